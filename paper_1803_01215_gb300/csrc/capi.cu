@@ -256,15 +256,6 @@ hj_status hj_solve_grad_unrolled(hj_problem prob, int64_t B, const double* xq, c
   if (xq == nullptr || t == nullptr || iters == nullptr || dL_dV == nullptr)
     return HJ_ERR_INVALID_ARG;
   const bool f64 = opts->precision == HJ_PREC_FP64;
-  const size_t tsz = f64 ? sizeof(double) : sizeof(float);
-  const int grid = hj::adjoint_grid(B);
-  const size_t per_cta = (size_t)(max_iters / checkpoint_every + 1) * 3 * (N + 1) * prob->d * tsz;
-  void* work = nullptr;
-  if (cudaMalloc(&work, per_cta * grid) != cudaSuccess) return HJ_ERR_OOM;
-  if (cudaMemsetAsync(prob->counter, 0, sizeof(unsigned long long), s) != cudaSuccess) {
-    cudaFree(work);
-    return HJ_ERR_CUDA;
-  }
   hj_status r;
   auto fill = [&](auto& a) {
     a.B = B; a.N = N; a.d = prob->d; a.K_cap = max_iters; a.C = checkpoint_every;
@@ -278,17 +269,13 @@ hj_status hj_solve_grad_unrolled(hj_problem prob, int64_t B, const double* xq, c
     hj::AdjArgs<double> a{};
     fill(a);
     a.sig = opts->sigma; a.tau = opts->tau; a.th = opts->theta;
-    a.work = static_cast<double*>(work);
-    r = hj::launch_adjoint<double>(prob->family, a, grid, s);
+    r = hj::launch_adjoint<double>(prob->family, a, s);
   } else {
     hj::AdjArgs<float> a{};
     fill(a);
     a.sig = (float)opts->sigma; a.tau = (float)opts->tau; a.th = (float)opts->theta;
-    a.work = static_cast<float*>(work);
-    r = hj::launch_adjoint<float>(prob->family, a, grid, s);
+    r = hj::launch_adjoint<float>(prob->family, a, s);
   }
-  if (cudaStreamSynchronize(s) != cudaSuccess && r == HJ_OK) r = HJ_ERR_CUDA;
-  cudaFree(work);
   return r;
 }
 
