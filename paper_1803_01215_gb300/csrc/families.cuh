@@ -77,6 +77,28 @@ __device__ __forceinline__ void v_fma(T (&r)[D], T s, const T (&x)[D], const T (
   for (int k = k0; k < D; ++k) r[k] = fma(s, x[k], y[k]);
 }
 
+// r = s * x + y on the coordinates k >= FROM, where x may be nonzero; r = y below
+template <int FROM, typename T, int D>
+__device__ __forceinline__ void v_fma_from(T (&r)[D], T s, const T (&x)[D], const T (&y)[D]) {
+  constexpr int F0 = sizeof(T) == 4 ? FROM + FROM % 2 : FROM;   // pairs from the next even coordinate
+  int k0 = F0;
+#pragma unroll
+  for (int k = 0; k < FROM; ++k) r[k] = y[k];
+#pragma unroll
+  for (int k = FROM; k < F0; ++k) r[k] = fma(s, x[k], y[k]);
+  if constexpr (sizeof(T) == 4) {
+#pragma unroll
+    for (int k = F0; k + 1 < D; k += 2) {
+      const float2 o = __ffma2_rn(make_float2(s, s), make_float2(x[k], x[k + 1]),
+                                  make_float2(y[k], y[k + 1]));
+      r[k] = o.x; r[k + 1] = o.y;
+    }
+    k0 = D - (D - F0) % 2;
+  }
+#pragma unroll
+  for (int k = k0; k < D; ++k) r[k] = fma(s, x[k], y[k]);
+}
+
 // r = s * x - y
 template <typename T, int D>
 __device__ __forceinline__ void v_fms(T (&r)[D], T s, const T (&x)[D], const T (&y)[D]) {
@@ -114,6 +136,10 @@ __device__ __forceinline__ T v_sumsq(const T (&e)[D]) {
   return acc;
 }
 
+// a b rounded once, never contracted with a following addition
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
 // a / b; FP32 uses the fast reciprocal-based division (2 ulp).
 template <typename T>
 __device__ __forceinline__ T fdiv(T a, T b) { return a / b; }
@@ -133,12 +159,13 @@ __device__ __forceinline__ float exp_t<float>(float y) { return __expf(y); }
 template <typename T>
 __device__ __forceinline__ T sqrt_t(T y) { return sqrt(y); }
 template <>
-__device__ __forceinline__ float sqrt_t<float>(float y) { return sqrtf(y); }
+__device__ __forceinline__ float sqrt_t<float>(float y) { return sqrt_rn_nb(y); }
 
 
 // ---------------------------------------------------------------- H = |p|^2/2
 template <typename T, int D>
 struct FamQuadratic {
+  static constexpr bool kBranchFree = true;    // a lane without a node may run the step
   static constexpr bool kHasGradX = false;
   static constexpr bool kGame = false;
   static constexpr bool kTimeDep = false;
@@ -198,7 +225,9 @@ struct FamQuadratic {
 template <typename T, int D>
 struct FamQuadcopter {
   static_assert(D == 12, "quadcopter state is 12-D");
+  static constexpr bool kBranchFree = true;    // a lane without a node may run the step
   static constexpr bool kHasGradX = true;
+  static constexpr int kGradFrom = 3;            // H does not depend on the position
   static constexpr bool kKktInIterType = true;   // kkt_node: FP32 iterates in FP32
   static constexpr bool kGame = false;
   static constexpr bool kTimeDep = false;
@@ -234,8 +263,27 @@ struct FamQuadcopter {
     J[8] = -cth * sph;
   }
 
+  // FP32: thrust's operations two-wide where they pair up, every fused form as the
+  // scalar code fuses it (J[0] = -a[1]).
   __device__ __forceinline__ void context(const T (&x)[D], Ctx& c) const {
-    thrust<T>(x[3], x[4], x[5], c.a, c.J);
+    if constexpr (sizeof(T) == 4) {
+      float sps, cps, sth, cth, sph, cph;
+      sin_cos<T>(x[3], &sps, &cps);
+      sin_cos<T>(x[4], &sth, &cth);
+      sin_cos<T>(x[5], &sph, &cph);
+      const float2 cc = __fmul2_rn(make_float2(cph, cph), make_float2(cps, sps));    // cc, cs
+      const float2 ss = __fmul2_rn(make_float2(sph, sph), make_float2(sps, -cps));   // ss, -sc
+      const float2 st = make_float2(sth, sth);
+      const float2 a01 = __ffma2_rn(cc, st, ss);
+      const float2 j14 = __fmul2_rn(cc, make_float2(cth, cth));
+      const float2 j52 = __ffma2_rn(ss, st, cc);                                     // -J5, J2
+      c.a[0] = a01.x; c.a[1] = a01.y; c.a[2] = cth * cph;
+      c.J[0] = -a01.y; c.J[1] = j14.x; c.J[2] = j52.y;
+      c.J[3] = a01.x;  c.J[4] = j14.y; c.J[5] = -j52.x;
+      c.J[6] = T(0);   c.J[7] = -sth * cph; c.J[8] = -cth * sph;
+    } else {
+      thrust<T>(x[3], x[4], x[5], c.a, c.J);
+    }
   }
 
   // Per-point constants of the prox: al = 1 + lam eps and the reciprocals used below.
@@ -257,7 +305,7 @@ struct FamQuadcopter {
                                        T (&v)[D]) const {
     const T lam = pc.lam, ial = pc.ial;
     if constexpr (sizeof(T) == 4) {
-      // rows 0-5: (v - lam x_{6..11}) * ial, rows 9-10 scaled, two-wide
+      // rows 0-5: (v - lam x_{6..11}) * ial, rows 10-11 scaled, two-wide
 #pragma unroll
       for (int k = 0; k < 6; k += 2) {
         const float2 t = __ffma2_rn(make_float2(-lam, -lam), make_float2(x[6 + k], x[7 + k]),
@@ -265,9 +313,23 @@ struct FamQuadcopter {
         const float2 o = __fmul2_rn(t, make_float2(ial, ial));
         v[k] = o.x; v[k + 1] = o.y;
       }
-      const float2 r = __fmul2_rn(make_float2(v[9], v[10]), make_float2(pc.irate, pc.irate));
-      v[9] = r.x; v[10] = r.y;
-      v[11] *= pc.irate;
+      // (10, 11) is a register pair of a 16-byte slot vector, (9, 10) is not
+      v[9] *= pc.irate;
+      const float2 r = __fmul2_rn(make_float2(v[10], v[11]), make_float2(pc.irate, pc.irate));
+      v[10] = r.x; v[11] = r.y;
+      // rows 6-8 as in the scalar form below, rows 6 and 7 two-wide
+      const float2 a01 = make_float2(c.a[0], c.a[1]);
+      const float2 w01 = __ffma2_rn(make_float2(-pc.lam_ah, -pc.lam_ah), a01, make_float2(v[6], v[7]));
+      const float w2 = v[8] - fmaf(pc.lam_ah, c.a[2], -pc.lam_gz);
+      const float2 b01 = __fmul2_rn(a01, make_float2(m_inv, m_inv));
+      const float b2 = c.a[2] * m_inv;
+      const float bb = fmaf(b2, b2, fmaf(b01.x, b01.x, __fmul_rn(b01.y, b01.y)));
+      const float bw = fmaf(b2, w2, fmaf(b01.x, w01.x, __fmul_rn(b01.y, w01.y)));
+      const float nf = fdiv<T>(-lam * bw, fmaf(lam, bb, pc.al));
+      const float2 o = __fmul2_rn(__ffma2_rn(make_float2(nf, nf), b01, w01), make_float2(ial, ial));
+      v[6] = o.x; v[7] = o.y;
+      v[8] = fmaf(nf, b2, w2) * ial;
+      return;
     } else {
 #pragma unroll
       for (int k = 0; k < 3; ++k) v[k] = (v[k] - lam * x[6 + k]) * ial;
@@ -393,12 +455,14 @@ struct FamQuadcopter {
 
   __device__ __forceinline__ void gradx(const Ctx& c, const T (&)[D], const T (&p)[D],
                                         T (&g)[D]) const {
-    const T u0 = (c.a[0] * p[6] + c.a[1] * p[7] + c.a[2] * p[8]) * m_inv;
-    const T coef = ah + u0 * m_inv;
+    // each dot product of three as fma(., ., fma(first, mul(second))), J[6] = 0
+    const T u0 = fma(c.a[2], p[8], fma(c.a[0], p[6], mul_rn(c.a[1], p[7]))) * m_inv;
+    const T coef = fma(u0, m_inv, ah);
     g[0] = g[1] = g[2] = T(0);
+    g[3] = coef * fma(c.J[0], p[6], mul_rn(c.J[3], p[7]));
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
-      g[3 + k] = coef * (c.J[k] * p[6] + c.J[3 + k] * p[7] + c.J[6 + k] * p[8]);
+    for (int k = 1; k < 3; ++k)
+      g[3 + k] = coef * fma(c.J[6 + k], p[8], fma(c.J[k], p[6], mul_rn(c.J[3 + k], p[7])));
 #pragma unroll
     for (int k = 0; k < 3; ++k) g[6 + k] = p[k];
 #pragma unroll
@@ -521,6 +585,7 @@ struct FamQuadcopter {
 // H = <p, tanh(A x)> + |p|^2/2; A is held in shared memory (broadcast reads).
 template <typename T, int D>
 struct FamTanhDrift {
+  static constexpr bool kBranchFree = true;    // a lane without a node may run the step
   static constexpr bool kHasGradX = true;
   static constexpr bool kGame = false;
   static constexpr bool kTimeDep = false;
@@ -634,6 +699,7 @@ struct FamTanhDrift {
 // time-aware members (context_t, Ht_t, H64_t) with s = j delta.
 template <typename T, int D, bool MOVING>
 struct FamEikonalT {
+  static constexpr bool kBranchFree = false;
   static constexpr bool kHasGradX = true;
   static constexpr bool kGame = false;
   static constexpr bool kTimeDep = MOVING;
@@ -769,8 +835,22 @@ using FamEikonalMoving = FamEikonalT<T, D, true>;
 // and its mirror c2(z) = c1(-z).  Both dual steps are shrink_2 (thresholds
 // lam c1 and lam c2); the primal step is game_step: a descent step for x at z^k,
 // then an ascent step for y at (x^{k+1}, y^k) (Algorithm 3's order).
-template <typename T, int D>
-struct FamGame {
+// D1 > 0: the minimiser's coordinate count d1 fixed at compile time (the paper's
+// games have d1 = 1), so every k < d1 folds; D1 = 0 takes it from the problem.
+template <int D1>
+struct GameSplit {
+  static constexpr int d1 = D1;
+  __device__ explicit GameSplit(int) {}
+};
+template <>
+struct GameSplit<0> {
+  int d1;
+  __device__ explicit GameSplit(int d1_) : d1(d1_) {}
+};
+template <typename T, int D, int D1>
+struct FamGameT : GameSplit<D1> {
+  using GameSplit<D1>::d1;
+  static constexpr bool kBranchFree = false;
   static constexpr bool kHasGradX = true;
   static constexpr bool kGame = true;
   static constexpr bool kTimeDep = false;
@@ -779,14 +859,13 @@ struct FamGame {
   struct PC { T lam; };
   const T* zb;
   const double* zb64;
-  int d1;
   T c0, am, bw;
   double c0d, amd, bwd;
   __device__ static void load_shared(const SolveArgs<T>& s, Shared& sh) {
     for (int i = threadIdx.x; i < D; i += blockDim.x) sh.zb[i] = s.xb[i];
   }
-  __device__ FamGame(const SolveArgs<T>& s, const Shared& sh)
-      : zb(sh.zb), zb64(s.xb64), d1(s.game_d1), c0(s.eik_t[0]), am(s.eik_t[1]),
+  __device__ FamGameT(const SolveArgs<T>& s, const Shared& sh)
+      : GameSplit<D1>(s.game_d1), zb(sh.zb), zb64(s.xb64), c0(s.eik_t[0]), am(s.eik_t[1]),
         bw(s.eik_t[2]), c0d(s.eik_c0), amd(s.eik_c1), bwd(s.eik_c2) {}
   __device__ __forceinline__ PC point(T lam) const { return PC{lam}; }
   __device__ __forceinline__ void context(const T (&z)[D], Ctx& c) const {
@@ -807,8 +886,8 @@ struct FamGame {
     T sp = T(0), sq = T(0);
 #pragma unroll
     for (int k = 0; k < D; ++k) {
-      if (k < d1) sp += P[k] * P[k];
-      else sq += P[k] * P[k];
+      if (k < d1) sp = fma(P[k], P[k], sp);
+      else sq = fma(P[k], P[k], sq);
     }
     np = sqrt_t<T>(sp);
     nq = sqrt_t<T>(sq);
@@ -912,5 +991,10 @@ struct FamGame {
     return c.c1 * np - c.c2 * nq;
   }
 };
+
+template <typename T, int D>
+using FamGame = FamGameT<T, D, 0>;
+template <typename T, int D>
+using FamGameOne = FamGameT<T, D, 1>;
 
 }  // namespace hj

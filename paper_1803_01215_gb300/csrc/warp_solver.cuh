@@ -92,6 +92,12 @@ template <class F>
 struct hopf_table<F, std::void_t<decltype(F::kHopfTable)>>
     : std::integral_constant<bool, F::kHopfTable> {};
 
+// first coordinate at which the family's grad_x H can be nonzero (F::kGradFrom)
+template <class F, class = void>
+struct grad_from : std::integral_constant<int, 0> {};
+template <class F>
+struct grad_from<F, std::void_t<decltype(F::kGradFrom)>> : std::integral_constant<int, F::kGradFrom> {};
+
 // lanes of this thread's 16-lane half
 __device__ __forceinline__ unsigned half_mask() { return 0xFFFFu << (threadIdx.x & 16); }
 
@@ -265,6 +271,20 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
   if constexpr (MIX) { if (own0) x0xslot[k0] = x0; }
   constexpr int DP = WarpShared<T, F, D, G, MIX, HOPF>::DP;
   constexpr int kLanes = group_lanes<G>();
+  // FP32, one node per lane, up to two warps per point (so that no warp is without a
+  // node), families without a root (F::kBranchFree): the steps run without
+  // branches on the node's index.  A lane past node N iterates on values that no other
+  // lane reads (node N's lane takes its own p for p_{N+1}); x_j stays where it is for
+  // j >= N because p_j - p_{j+1} and the gradient's factor are zero there.  With the
+  // rows and angles of the quadcopter two-wide and two iterations per trip the loop
+  // went from 190 to 165 instructions per warp and iteration (64 % of the FMA pipe's
+  // cycles, as before, are what holds a full GPU): N = 64, FP32, B = 4096 2.34 -> 2.20 ms,
+  // B = 1 288 -> 245 us.  20 or more warps per SM (85 registers, no spills) ran 5 %
+  // slower; families whose idle lanes would take a root's rare path, and larger groups,
+  // keep the guards (a guard per warp instead ran the batch 6 % slower).
+  constexpr bool kFree = NPL == 1 && G <= 2 && sizeof(T) == 4 && F::kBranchFree;
+  [[maybe_unused]] const int pr_lane = jbase < N ? gl + 1 : gl;
+  const T taud_x = (!kFree || jbase < N) ? taud : T(0);
 
   // One iteration; CHK adds the squared increments (test iterations only, so
   // the plain iterations carry no residual code at all).
@@ -281,6 +301,8 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
   auto step = [&](auto chk_tag, T& rx, T& rp, T& vacc) {
     constexpr bool CHK = decltype(chk_tag)::value;
     typename F::Ctx ctx[NPL];
+    // H's quantities at x^k before the exchange: independent work for its latency
+    if constexpr (kFree) node_context(fam, x[0], T(jbase) * delta_t, ctx[0]);
     // ---- z_{j-1} of the first owned node: the left lane's slot (z^k of its last node)
     slot_store<T, D>(zslot + gl * DP, z[NPL - 1]);
     if constexpr (MIX) slot_store<T, D>(xslot + gl * DP, x[NPL - 1]);
@@ -299,8 +321,8 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
     }
 #pragma unroll
     for (int i = 0; i < NPL; ++i) {
-      if (jbase + i <= N) {
-        node_context(fam, x[i], T(jbase + i) * delta_t, ctx[i]);
+      if (kFree || jbase + i <= N) {
+        if constexpr (!kFree) node_context(fam, x[i], T(jbase + i) * delta_t, ctx[i]);
         T v[D], dz[D];
         if (i == 0) v_sub<T, D>(dz, z[i], zl);
         else v_sub<T, D>(dz, z[i], z[i > 0 ? i - 1 : 0]);
@@ -322,7 +344,8 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
         if constexpr (CHK) {
           T e[D];
           v_sub<T, D>(e, v, p[i]);
-          rp += v_sumsq<T, D>(e);
+          const T s2 = v_sumsq<T, D>(e);
+          rp += (!kFree || jbase + i <= N) ? s2 : T(0);
         }
 #pragma unroll
         for (int k = 0; k < D; ++k) p[i][k] = v[k];
@@ -341,15 +364,13 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
     // ---- primal step: p_{j+1} of the last owned node from the right lane's slot
     slot_store<T, D>(pslot + gl * DP, p[0]);
     group_sync<G>();
+    // (kFree: a lane without an x update reads its own slot, so that p_j - p_{j+1} is 0;
+    // else the last lane never updates an x with what it reads)
     T pr[D];
-    if (gl + 1 < kLanes) {
-      slot_load<T, D>(pslot + (gl + 1) * DP, pr);
-    } else {
-#pragma unroll
-      for (int k = 0; k < D; ++k) pr[k] = T(0);    // the last lane never updates an x with it
-    }
-    if (own0 && !HOPF) {
+    slot_load<T, D>(pslot + (kFree ? pr_lane : (gl + 1 < kLanes ? gl + 1 : gl)) * DP, pr);
+    if ((own0 || (kFree && !MIX)) && !HOPF) {
       // x_0 <- prox_{tau g}(x_0 + tau p_1), coordinate k0; p_1 is lane 0's slot
+      // (a lane that owns no coordinate repeats coordinate 0's arithmetic)
       T xn;
       if constexpr (MIX && F::kGame) {
         // the whole node-0 step in every x_0 lane (the y-block needs all of x_0^{k+1})
@@ -367,21 +388,21 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
         }
         xn = (v0 + goff) * ginv;
       }
-      if constexpr (CHK) { const T e = xn - x0; rx += e * e; }
+      if constexpr (CHK) { const T e = xn - x0; rx += own0 ? e * e : T(0); }
       if constexpr (CHK && kValueTest) {
-        if (a.value_stop) {                              // g(x_0) - <p_1, x_0>, coordinate k0
+        if (a.value_stop && own0) {                      // g(x_0) - <p_1, x_0>, coordinate k0
           const T e = xn - T(sh.cd[k0]);
           vacc += T(0.5) * T(sh.w2d[k0]) * e * e - coord_sign(k0) * pslot[k0] * xn;
         }
       }
       z0 = relax<T, TH1>(xn, x0, th);
       x0 = xn;
-      x0slot[k0] = z0;
-      if constexpr (MIX) x0xslot[k0] = xn;
+      if (own0) x0slot[k0] = z0;
+      if constexpr (MIX) { if (own0) x0xslot[k0] = xn; }
     }
 #pragma unroll
     for (int i = 0; i < NPL; ++i) {
-      if (jbase + i < N) {
+      if (kFree || jbase + i < N) {
         T xn[D], dp[D];
         if (i == NPL - 1) v_sub<T, D>(dp, p[i], pr);
         else v_sub<T, D>(dp, p[i], p[i + 1 < NPL ? i + 1 : i]);
@@ -392,9 +413,9 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
           fam.norms(p[i], np1, nq1);
           if (i == NPL - 1) fam.norms(pr, np2, nq2);
           else fam.norms(p[i + 1 < NPL ? i + 1 : i], np2, nq2);
-          fam.game_step_norms(ctx[i], x[i], wr * np1 + wl * np2, wr * nq1 + wl * nq2, taud, xn);
+          fam.game_step_norms(ctx[i], x[i], wr * np1 + wl * np2, wr * nq1 + wl * nq2, taud_x, xn);
         } else if constexpr (F::kGame) {
-          fam.game_step(ctx[i], x[i], p[i], taud, xn);      // descent in x, ascent in y
+          fam.game_step(ctx[i], x[i], p[i], taud_x, xn);      // descent in x, ascent in y
         } else if constexpr (MIX) {
           // + tau delta (wR grad_x H(x_j, p_j) + wL grad_x H(x_j, p_{j+1}))
           T g[D], g2[D];
@@ -406,19 +427,19 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
           T base[D];
 #pragma unroll
           for (int k = 0; k < D; ++k) base[k] = xn[k];
-          v_fma<T, D>(xn, taud, g, base);
+          v_fma<T, D>(xn, taud_x, g, base);
         } else if (F::kHasGradX) {
           T g[D];
           fam.gradx(ctx[i], x[i], p[i], g);
           T base[D];
 #pragma unroll
           for (int k = 0; k < D; ++k) base[k] = xn[k];
-          v_fma<T, D>(xn, taud, g, base);                    // + tau delta grad_x H
+          v_fma_from<grad_from<F>::value, T, D>(xn, taud_x, g, base);   // + tau delta grad_x H
           for (int s = 1; s < a.inner_steps; ++s) {
             typename F::Ctx c2;
             node_context(fam, xn, T(jbase + i) * delta_t, c2);
             fam.gradx(c2, xn, p[i], g);
-            v_fma<T, D>(xn, taud, g, base);
+            v_fma<T, D>(xn, taud_x, g, base);
           }
         }
         if constexpr (CHK) {
@@ -427,7 +448,7 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
           rx += v_sumsq<T, D>(e);
         }
         if constexpr (CHK && kValueTest) {
-          if (a.value_stop) {                            // <p_j - p_{j+1}, x_j> - delta H(x_j, p_j)
+          if (a.value_stop && (!kFree || jbase + i < N)) {  // <p_j - p_{j+1}, x_j> - delta H(x_j, p_j)
             T s = T(0);
 #pragma unroll
             for (int k = 0; k < D; ++k) s += coord_sign(k) * dp[k] * xn[k];
@@ -442,7 +463,8 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
         }
 #pragma unroll
         for (int k = 0; k < D; ++k) x[i][k] = xn[k];
-      } else if (jbase + i == N) {
+      }
+      if (jbase + i == N) {
         if constexpr (CHK && kValueTest) {
           if (a.value_stop) {                            // <p_N, x_N> - delta H(x_N, p_N)
             T s = T(0);
@@ -465,6 +487,9 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
     const int left = max_iter - k_it;
     const int plain = (check_every - 1 < left - 1) ? check_every - 1 : left - 1;
     T dummy_x = T(0), dummy_p = T(0), dummy_v = T(0);
+    // two iterations per trip (FP32, branch-free step): the new x of one is the old x
+    // of the next, so fewer registers are copied at the loop's end
+#pragma unroll (kFree ? 2 : 1)
     for (int r = 0; r < plain; ++r)
       step(std::integral_constant<bool, false>{}, dummy_x, dummy_p, dummy_v);
     T rx = T(0), rp = T(0), vacc = T(0);
@@ -504,6 +529,12 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
   }
 
   // ---- value (fval of Algorithm 1), summed in FP64, and outputs
+  if constexpr (kFree) {
+    // x_N = x whatever the iteration did to it (0 * an infinite p is not 0)
+    if (jbase == N)
+#pragma unroll
+      for (int k = 0; k < D; ++k) x[0][k] = T(pt.xq[k]);
+  }
   group_sync<G>();                                 // every lane is done with the slots
   slot_store<T, D>(zslot + gl * DP, x[NPL - 1]);
   if (own0) x0slot[k0] = x0;
@@ -522,7 +553,8 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
           T s = T(0);
 #pragma unroll
           for (int k = 0; k < D; ++k) {
-            const T term = p[i][k] * (x[i][k] - ((i == 0) ? xl[k] : x[i - 1][k]));
+            const T dxk = x[i][k] - ((i == 0) ? xl[k] : x[i - 1][k]);
+            const T term = F::kGame ? mul_rn(p[i][k], dxk) : p[i][k] * dxk;
             if constexpr (F::kGame) s += (k < fam.d1) ? term : -term;   // <p, dx> - <q, dy>
             else s += term;
           }
@@ -537,7 +569,8 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
 #pragma unroll
           for (int k = 0; k < D; ++k) {
             const double xm = (double)((i == 0) ? xl[k] : x[i - 1][k]);
-            const double term = (double)p[i][k] * ((double)x[i][k] - xm);
+            const double dxk = (double)x[i][k] - xm;
+            const double term = F::kGame ? mul_rn((double)p[i][k], dxk) : (double)p[i][k] * dxk;
             if constexpr (F::kGame) s += (k < fam.d1) ? term : -term;
             else s += term;
           }
