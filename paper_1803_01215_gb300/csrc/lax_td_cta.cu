@@ -17,6 +17,14 @@
 // the iterate type, over the warps as double-floats or in FP64).  CTAs
 // draw points from a work counter (persistent grid).
 //
+// FP64 iterates are bound by the FP64 pipe (80 % busy: one instruction holds a
+// sub-partition's pipe about 64 cycles per warp), so what counts is the FP64
+// instructions per element: 70 of them were CUDA's tanh (both of its ranges, for a warp
+// whose lanes differ), 14 are the Taylor table's (tanh64.cuh); and for N a multiple of
+// 4 the tiles start at node 1 (node_shift): at d = N = 32 two whole warps of tiles
+// instead of two and a quarter, which cost three.
+// d = N = 32, 512 points, FP64: 86.4 -> 56.5 ms.
+//
 // MIX = true runs the forward-Euler and trapezoid schemes (HJ_SCHEME_FE/TRAP),
 // H on interval j weighted wR at x_j and wL at x_{j-1}: phase A stores
 // a = tanh(A x) for every node 0..N in a fifth state array, the dual step
@@ -26,6 +34,7 @@
 #include <cuda_runtime.h>
 
 #include "hj_internal.cuh"
+#include "tanh64.cuh"
 
 namespace hj {
 
@@ -55,9 +64,18 @@ struct Vec4<double> {
 __host__ __device__ inline int round4(int v) { return (v + 3) & ~3; }
 
 template <typename T>
-__device__ __forceinline__ T tanh_c(T y) { return tanh(y); }
+__device__ __forceinline__ T tanh_c(T y, const double* tab);
 template <>
-__device__ __forceinline__ float tanh_c<float>(float y) { return tanhf(y); }
+__device__ __forceinline__ double tanh_c<double>(double y, const double* tab) {
+  return tab != nullptr ? tanh_taylor(y, tab) : tanh(y);
+}
+template <>
+__device__ __forceinline__ float tanh_c<float>(float y, const double*) { return tanhf(y); }
+
+// Node j of a point with N steps is column j + node_shift(N) of the state arrays: for
+// N a multiple of 4 the nodes 1..N fill whole 4-column tiles and node 0 sits in the
+// last column of a tile of its own (the products skip it, mixed schemes apart).
+__host__ __device__ inline int node_shift(int N) { return N % 4 == 0 ? 3 : 0; }
 
 struct Layout {
   int dp, Np;               // padded coordinate count and node count
@@ -73,7 +91,8 @@ struct Layout {
 
 // TWO: keep both A^T and A in shared memory (vector loads in both products);
 // otherwise only A, and the first product reads it with strided scalar loads.
-template <typename T, bool TWO, bool DRIFT, bool HOPF, bool MIX>
+// TAB: tanh of FP64 iterates from the Taylor table, kept in shared memory.
+template <typename T, bool TWO, bool DRIFT, bool HOPF, bool MIX, bool TAB>
 __global__ void __launch_bounds__(512)
 lax_td_cta_kernel(const SolveArgs<T> a) {
   static_assert(!(MIX && (HOPF || !DRIFT)), "the mixed schemes: Lax form, tanh drift");
@@ -92,6 +111,7 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
   double* tred = red;                                       // [2 * nwarps] stopping test
   T* hsv = reinterpret_cast<T*>(red + 32);                  // Hopf form: sigma / W^2, sigma c
   T* hcv = hsv + dp;
+  double* ttab = TAB ? reinterpret_cast<double*>(hcv + dp) : nullptr;   // 16-byte aligned: every part above is
   __shared__ unsigned long long s_point;
 
   const int tid = threadIdx.x, nthr = blockDim.x;
@@ -109,6 +129,7 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
     hsv[i] = (HOPF && i < d) ? T(a.sigma / a.W2[i]) : T(0);
     hcv[i] = (i < d) ? T(a.sigma * a.c[i]) : T(0);
   }
+  if constexpr (TAB) tanh_taylor_table(ttab, tid, nthr);
   const T sig = a.sigma_t, tau = a.tau_t, th = a.theta_t;
   const T wr = a.mix_wr_t, wl = a.mix_wl_t;
 
@@ -126,7 +147,9 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
       continue;
     }
     const int Np = round4(N + 1);
-    const int tilesI = dp / kTI, tilesJ = Np / kTJ;
+    const int sh = node_shift(N);                          // node j: column j + sh
+    const int jt0 = (sh > 0 && !MIX) ? 1 : 0;              // first tile the products run on
+    const int tilesI = dp / kTI, tilesJ = Np / kTJ - jt0;
     const int ntiles = tilesI * tilesJ;
     const double delta = a.t[b] / N;                      // value epilogue only
     const T delta_t = T(a.t[b]) / T(N);
@@ -136,9 +159,9 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
 
     // ---- initial iterate (Section 6 random guess, or a warm start)
     for (int e = tid; e < dp * Np; e += nthr) {
-      const int k = e / Np, j = e - k * Np;
+      const int k = e / Np, j = e - k * Np - sh;
       T xv = T(0), pv = T(0);
-      if (k < d && j <= N && !(HOPF && j == 0)) {         // Hopf: x_0 is not a variable (0)
+      if (k < d && j >= 0 && j <= N && !(HOPF && j == 0)) {         // Hopf: x_0 is not a variable (0)
         const double xq = ref.xq[k];
         if (a.warm_x == nullptr) {
           const InitGuess<T> ig(a.radius);
@@ -161,7 +184,7 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
       T rx = T(0), rp = T(0);
       // ---- phase A: Y = A X, tanh, dual prox, W = (1 - a^2) p
       for (int tile = tid; tile < ntiles; tile += nthr) {
-        const int i0 = (tile % tilesI) * kTI, j0 = (tile / tilesI) * kTJ;
+        const int i0 = (tile % tilesI) * kTI, j0 = (jt0 + tile / tilesI) * kTJ;   // j0: a column
         T acc[kTI][kTJ];
 #pragma unroll
         for (int r = 0; r < kTI; ++r)
@@ -187,17 +210,17 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
           for (int r = 0; r < kTI; ++r)
 #pragma unroll
             for (int c = 0; c < kTJ; ++c)
-              if (i0 + r < d && j0 + c <= N) Asv[(i0 + r) * Np + j0 + c] = tanh_c<T>(acc[r][c]);
+              if (i0 + r < d && j0 + c <= N + sh) Asv[(i0 + r) * Np + j0 + c] = tanh_c<T>(acc[r][c], ttab);
         } else {
 #pragma unroll
         for (int r = 0; r < kTI; ++r) {
           const int i = i0 + r;
 #pragma unroll
           for (int c = 0; c < kTJ; ++c) {
-            const int j = j0 + c;
+            const int j = j0 + c - sh;
             if (i < d && j >= 1 && j <= N) {
-              const int e = i * Np + j;
-              const T av = DRIFT ? tanh_c<T>(acc[r][c]) : T(0);
+              const int e = i * Np + j0 + c;
+              const T av = DRIFT ? tanh_c<T>(acc[r][c], ttab) : T(0);
               const T v = P[e] + sig * (Z[e] - Z[e - 1]);
               const T pn = (HOPF && j == 1)         // Hopf node 1: prox of sigma g* + lam H
                                ? (v - hcv[i] - lam * av) / (T(1) + lam + hsv[i])
@@ -215,7 +238,7 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
         // dual step with the averaged drift: (1 + lam) p = v - lam (wR a_j + wL a_{j-1})
         for (int e2 = tid; e2 < d * N; e2 += nthr) {
           const int i = e2 / N, j = 1 + (e2 - i * N);
-          const int e = i * Np + j;
+          const int e = i * Np + j + sh;
           const T v = P[e] + sig * (Z[e] - Z[e - 1]);
           const T pn = (v - lam * (wr * Asv[e] + wl * Asv[e - 1])) * ilam;
           if (chk) { const T df = pn - P[e]; rp += df * df; }
@@ -225,7 +248,7 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
         // W = (1 - a_j^2)(wR p_j + wL p_{j+1}), j = 1..N-1; node 0: wL (1 - a_0^2) p_1
         for (int e2 = tid; e2 < d * N; e2 += nthr) {
           const int i = e2 / N, j = e2 - i * N;
-          const int e = i * Np + j;
+          const int e = i * Np + j + sh;
           const T av = Asv[e];
           const T pw = (j == 0) ? wl * P[e + 1] : wr * P[e] + wl * P[e + 1];
           Wk[e] = (T(1) - av * av) * pw;
@@ -234,7 +257,7 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
       __syncthreads();
       // ---- phase B: G = A^T W, primal gradient step, relaxation; g-prox of x_0
       for (int tile = tid; tile < ntiles; tile += nthr) {
-        const int i0 = (tile % tilesI) * kTI, j0 = (tile / tilesI) * kTJ;
+        const int i0 = (tile % tilesI) * kTI, j0 = (jt0 + tile / tilesI) * kTJ;   // j0: a column
         T acc[kTI][kTJ];
 #pragma unroll
         for (int r = 0; r < kTI; ++r)
@@ -255,9 +278,9 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
           const int i = i0 + r;
 #pragma unroll
           for (int c = 0; c < kTJ; ++c) {
-            const int j = j0 + c;
+            const int j = j0 + c - sh;
             if (i < d && j >= 1 && j < N) {
-              const int e = i * Np + j;
+              const int e = i * Np + j0 + c;
               const T xo = X[e];
               const T xn = xo - tau * (P[e] - P[e + 1]) + taud * acc[r][c];
               if (chk) { const T df = xn - xo; rx += df * df; }
@@ -265,7 +288,7 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
               X[e] = xn;
             } else if (MIX && i < d && j == 0) {
               // x_0: gradient step on -delta wL H(x_0, p_1) (in W), then the prox of g
-              const int e = i * Np;
+              const int e = i * Np + sh;
               const T w2 = T(a.W2[i]), cc = T(a.c[i]);
               const T xo = X[e];
               const T xn = (xo + tau * P[e + 1] + taud * acc[r][c] + tau * w2 * cc) /
@@ -278,7 +301,7 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
         }
       }
       if (!HOPF && !MIX && tid < d) {
-        const int e = tid * Np;
+        const int e = tid * Np + sh;
         const T w2 = T(a.W2[tid]), cc = T(a.c[tid]);
         const T xo = X[e];
         const T xn = (xo + tau * P[e + 1] + tau * w2 * cc) / (T(1) + tau * w2);
@@ -314,13 +337,13 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
         if (DRIFT) {
           T y = T(0), yl = T(0);
           for (int k = 0; k < d; ++k) {
-            y += Am[i * dp + k] * X[k * Np + j];
-            if (MIX) yl += Am[i * dp + k] * X[k * Np + j - 1];
+            y += Am[i * dp + k] * X[k * Np + j + sh];
+            if (MIX) yl += Am[i * dp + k] * X[k * Np + j - 1 + sh];
           }
-          th_y = MIX ? wr * tanh_c<T>(y) + wl * tanh_c<T>(yl) : tanh_c<T>(y);
+          th_y = MIX ? wr * tanh_c<T>(y, nullptr) + wl * tanh_c<T>(yl, nullptr) : tanh_c<T>(y, nullptr);
         }
-        const T pv = P[i * Np + j];
-        const T dx = X[i * Np + j] - X[i * Np + j - 1];
+        const T pv = P[i * Np + j + sh];
+        const T dx = X[i * Np + j + sh] - X[i * Np + j - 1 + sh];
         acc += (double)(pv * dx - delta_t * (pv * th_y + T(0.5) * pv * pv));
       } else {
         double th_y = 0.0;
@@ -328,22 +351,22 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
           const double* Ar = a.A64 + (size_t)i * d;
           double y = 0.0, yl = 0.0;
           for (int k = 0; k < d; ++k) {
-            y += Ar[k] * (double)X[k * Np + j];
-            if (MIX) yl += Ar[k] * (double)X[k * Np + j - 1];
+            y += Ar[k] * (double)X[k * Np + j + sh];
+            if (MIX) yl += Ar[k] * (double)X[k * Np + j - 1 + sh];
           }
           th_y = MIX ? a.mix_wr * tanh(y) + a.mix_wl * tanh(yl) : tanh(y);
         }
-        const double pv = (double)P[i * Np + j];
-        const double dx = (double)X[i * Np + j] - (double)X[i * Np + j - 1];
+        const double pv = (double)P[i * Np + j + sh];
+        const double dx = (double)X[i * Np + j + sh] - (double)X[i * Np + j - 1 + sh];
         acc += pv * dx - delta * (pv * th_y + 0.5 * pv * pv);
       }
     }
     if (tid < d) {
       if (HOPF) {                                         // -g*(p_1)
-        const double p1 = (double)P[tid * Np + 1];
+        const double p1 = (double)P[tid * Np + 1 + sh];
         acc -= p1 * a.c[tid] + 0.5 * p1 * p1 / a.W2[tid];
       } else {
-        const double e0 = (double)X[tid * Np] - a.c[tid];
+        const double e0 = (double)X[tid * Np + sh] - a.c[tid];
         acc += 0.5 * a.W2[tid] * e0 * e0;
       }
     }
@@ -364,9 +387,9 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
         const int j = e / d, i = e - j * d;
         if (a.traj_x != nullptr)                          // Hopf: x_0 = c + p_1 / W^2
           a.traj_x[ref.traj + e] = (HOPF && j == 0)
-                                       ? T(a.c[i] + (double)P[i * Np + 1] / a.W2[i])
-                                       : X[i * Np + j];
-        if (a.traj_p != nullptr) a.traj_p[ref.traj + e] = (j == 0) ? T(0) : P[i * Np + j];
+                                       ? T(a.c[i] + (double)P[i * Np + 1 + sh] / a.W2[i])
+                                       : X[i * Np + j + sh];
+        if (a.traj_p != nullptr) a.traj_p[ref.traj + e] = (j == 0) ? T(0) : P[i * Np + j + sh];
       }
     }
   }
@@ -380,9 +403,9 @@ size_t smem_bytes(int d, int N, bool drift, bool mix = false) {
          2 * 16 * sizeof(double);
 }
 
-template <typename T, bool TWO, bool DRIFT, bool HOPF, bool MIX>
-hj_status launch_form(const SolveArgs<T>& a, cudaStream_t s, size_t smem) {
-  auto kern = lax_td_cta_kernel<T, TWO, DRIFT, HOPF, MIX>;
+template <typename T, bool TWO, bool DRIFT, bool HOPF, bool MIX, bool TAB>
+hj_status launch_tab(const SolveArgs<T>& a, cudaStream_t s, size_t smem) {
+  auto kern = lax_td_cta_kernel<T, TWO, DRIFT, HOPF, MIX, TAB>;
   int dev = 0, nsm = 0, max_optin = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return HJ_ERR_CUDA;
   if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -395,7 +418,7 @@ hj_status launch_form(const SolveArgs<T>& a, cudaStream_t s, size_t smem) {
       cudaSuccess)
     return HJ_ERR_CUDA;
   const Layout L(a.d, a.N);
-  const int tiles = (L.dp / kTI) * (L.Np / kTJ);
+  const int tiles = (L.dp / kTI) * (L.Np / kTJ - ((node_shift(a.N) > 0 && !MIX) ? 1 : 0));
   int threads = ((tiles + 31) / 32) * 32;
   if (threads < 64) threads = 64;
   if (threads > 512) threads = 512;
@@ -408,6 +431,16 @@ hj_status launch_form(const SolveArgs<T>& a, cudaStream_t s, size_t smem) {
   const int grid = (int)(a.B < cap ? a.B : cap);
   kern<<<grid, threads, smem, s>>>(a);
   return cudaGetLastError() == cudaSuccess ? HJ_OK : HJ_ERR_CUDA;
+}
+
+// FP64 drift: the Taylor table wherever its 29 KB fit beside the state; CUDA's tanh elsewhere
+template <typename T, bool TWO, bool DRIFT, bool HOPF, bool MIX>
+hj_status launch_form(const SolveArgs<T>& a, cudaStream_t s, size_t smem) {
+  if constexpr (sizeof(T) == 8 && DRIFT) {
+    const size_t tab = smem + kTanhRows * kTanhRow * sizeof(double);
+    if (tab <= 227u * 1024u) return launch_tab<T, TWO, DRIFT, HOPF, MIX, true>(a, s, tab);
+  }
+  return launch_tab<T, TWO, DRIFT, HOPF, MIX, false>(a, s, smem);
 }
 
 template <typename T, bool TWO, bool DRIFT>
