@@ -23,7 +23,9 @@
 // whose lanes differ), 14 are the Taylor table's (tanh64.cuh); and for N a multiple of
 // 4 the tiles start at node 1 (node_shift): at d = N = 32 two whole warps of tiles
 // instead of two and a quarter, which cost three.
-// d = N = 32, 512 points, FP64: 86.4 -> 56.5 ms.
+// FP64 CTAs hold several groups with a point each, sharing A and the table, so that four
+// points instead of two fit an SM.  d = N = 32, 512 points, FP64: 86.4 -> 56.5 ms, with
+// the groups 52.2.
 //
 // MIX = true runs the forward-Euler and trapezoid schemes (HJ_SCHEME_FE/TRAP),
 // H on interval j weighted wR at x_j and wL at x_{j-1}: phase A stores
@@ -87,14 +89,19 @@ struct Layout {
     a_elems = (size_t)d * dp;
     s_elems = (size_t)dp * Np;
   }
+  // one group's state arrays and reduction scratch
+  __host__ __device__ size_t group_bytes(size_t elem, bool mix) const {
+    return (mix ? 5 : 4) * s_elems * elem + 2 * 16 * sizeof(double);
+  }
 };
+constexpr int kMaxGroups = 8;
 
 // TWO: keep both A^T and A in shared memory (vector loads in both products);
 // otherwise only A, and the first product reads it with strided scalar loads.
 // TAB: tanh of FP64 iterates from the Taylor table, kept in shared memory.
 template <typename T, bool TWO, bool DRIFT, bool HOPF, bool MIX, bool TAB>
 __global__ void __launch_bounds__(512)
-lax_td_cta_kernel(const SolveArgs<T> a) {
+lax_td_cta_kernel(const SolveArgs<T> a, int M) {
   static_assert(!(MIX && (HOPF || !DRIFT)), "the mixed schemes: Lax form, tanh drift");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int d = a.d;
@@ -102,23 +109,34 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
   const int dp = L.dp;
   T* Am = reinterpret_cast<T*>(smem_raw);                 // Am[k*dp + i] = A[k][i]
   T* At = TWO ? Am + L.a_elems : Am;                      // At[k*dp + i] = A[i][k]
-  T* X = DRIFT ? (TWO ? At + L.a_elems : Am + L.a_elems) : Am;   // no A without drift
+  T* hsv = DRIFT ? (TWO ? At + L.a_elems : Am + L.a_elems) : Am;  // no A without drift
+  T* hcv = hsv + dp;                                        // Hopf form: sigma / W^2, sigma c
+  double* ttab = TAB ? reinterpret_cast<double*>(hcv + dp) : nullptr;   // 16-byte aligned, as every part
+  // M groups of threads (TAB; else one), each with a point of its own
+  const int nthr = TAB ? (int)blockDim.x / M : (int)blockDim.x;
+  const int grp = TAB ? (int)threadIdx.x / nthr : 0;
+  const int tid = (int)threadIdx.x - grp * nthr;
+  T* X = reinterpret_cast<T*>(reinterpret_cast<unsigned char*>(hcv + dp) +
+                              (TAB ? kTanhRows * kTanhRow * sizeof(double) : 0) +
+                              grp * L.group_bytes(sizeof(T), MIX));
   T* P = X + L.s_elems;
   T* Z = P + L.s_elems;
   T* Wk = Z + L.s_elems;
   T* Asv = Wk + L.s_elems;                                  // MIX: tanh(A x) of every node
   double* red = reinterpret_cast<double*>(Wk + (MIX ? 2 : 1) * L.s_elems);  // [2 * nwarps]
   double* tred = red;                                       // [2 * nwarps] stopping test
-  T* hsv = reinterpret_cast<T*>(red + 32);                  // Hopf form: sigma / W^2, sigma c
-  T* hcv = hsv + dp;
-  double* ttab = TAB ? reinterpret_cast<double*>(hcv + dp) : nullptr;   // 16-byte aligned: every part above is
-  __shared__ unsigned long long s_point;
+  __shared__ unsigned long long s_points[kMaxGroups];
+  unsigned long long& s_point = s_points[grp];
+  // barrier of the group's threads
+  auto sync = [&]() {
+    if constexpr (TAB) asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(nthr) : "memory");
+    else __syncthreads();
+  };
 
-  const int tid = threadIdx.x, nthr = blockDim.x;
   const int warp = tid >> 5, lane = tid & 31, nwarps = nthr >> 5;
 
   if (DRIFT) {
-    for (int e = tid; e < d * dp; e += nthr) {
+    for (int e = threadIdx.x; e < d * dp; e += blockDim.x) {
       const int k = e / dp, i = e - k * dp;
       Am[e] = (i < d) ? a.A[k * d + i] : T(0);
       if (TWO) At[e] = (i < d) ? a.At[k * d + i] : T(0);
@@ -129,14 +147,15 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
     hsv[i] = (HOPF && i < d) ? T(a.sigma / a.W2[i]) : T(0);
     hcv[i] = (i < d) ? T(a.sigma * a.c[i]) : T(0);
   }
-  if constexpr (TAB) tanh_taylor_table(ttab, tid, nthr);
+  if constexpr (TAB) tanh_taylor_table(ttab, threadIdx.x, blockDim.x);
+  __syncthreads();
   const T sig = a.sigma_t, tau = a.tau_t, th = a.theta_t;
   const T wr = a.mix_wr_t, wl = a.mix_wl_t;
 
   for (;;) {
-    __syncthreads();
+    sync();
     if (tid == 0) s_point = draw_item(a);
-    __syncthreads();
+    sync();
     const int64_t item = (int64_t)s_point;
     if (item >= a.B) break;
     const PointRef<T> ref = point_ref(a, item);
@@ -174,7 +193,7 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
       }
       X[e] = xv; P[e] = pv; Z[e] = xv; Wk[e] = T(0);
     }
-    __syncthreads();
+    sync();
 
     int k_it = 0;
     int8_t st = HJ_POINT_MAX_ITER;
@@ -234,7 +253,7 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
         }
       }
       if constexpr (MIX) {
-        __syncthreads();
+        sync();
         // dual step with the averaged drift: (1 + lam) p = v - lam (wR a_j + wL a_{j-1})
         for (int e2 = tid; e2 < d * N; e2 += nthr) {
           const int i = e2 / N, j = 1 + (e2 - i * N);
@@ -244,7 +263,7 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
           if (chk) { const T df = pn - P[e]; rp += df * df; }
           P[e] = pn;
         }
-        __syncthreads();
+        sync();
         // W = (1 - a_j^2)(wR p_j + wL p_{j+1}), j = 1..N-1; node 0: wL (1 - a_0^2) p_1
         for (int e2 = tid; e2 < d * N; e2 += nthr) {
           const int i = e2 / N, j = e2 - i * N;
@@ -254,7 +273,7 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
           Wk[e] = (T(1) - av * av) * pw;
         }
       }
-      __syncthreads();
+      sync();
       // ---- phase B: G = A^T W, primal gradient step, relaxation; g-prox of x_0
       for (int tile = tid; tile < ntiles; tile += nthr) {
         const int i0 = (tile % tilesI) * kTI, j0 = (jt0 + tile / tilesI) * kTJ;   // j0: a column
@@ -317,7 +336,7 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
         const T wx = warp_sum<T>(rx), wp = warp_sum<T>(rp);
         if (lane == 0) { tsum[2 * warp] = wx; tsum[2 * warp + 1] = wp; }
       }
-      __syncthreads();
+      sync();
       if (chk) {
         const int verdict = stop_verdict<T>(a, tsum, nwarps, lane);   // 1 converged, 2 non-finite
         if (verdict == 2) { st = HJ_POINT_NONFINITE; break; }
@@ -371,9 +390,9 @@ lax_td_cta_kernel(const SolveArgs<T> a) {
       }
     }
     acc = warp_sum<double>(acc);
-    __syncthreads();
+    sync();
     if (lane == 0) red[warp] = acc;
-    __syncthreads();
+    sync();
     if (tid == 0) {
       double v = 0.0;
       for (int w = 0; w < nwarps; ++w) v += red[w];
@@ -399,8 +418,7 @@ template <typename T, bool TWO>
 size_t smem_bytes(int d, int N, bool drift, bool mix = false) {
   const Layout L(d, N);
   const size_t na = drift ? (TWO ? 2 : 1) : 0;
-  return (na * L.a_elems + (mix ? 5 : 4) * L.s_elems + 2 * L.dp) * sizeof(T) +
-         2 * 16 * sizeof(double);
+  return (na * L.a_elems + 2 * L.dp) * sizeof(T) + L.group_bytes(sizeof(T), mix);
 }
 
 template <typename T, bool TWO, bool DRIFT, bool HOPF, bool MIX, bool TAB>
@@ -414,22 +432,37 @@ hj_status launch_tab(const SolveArgs<T>& a, cudaStream_t s, size_t smem) {
       cudaSuccess)
     return HJ_ERR_CUDA;
   if (smem > (size_t)max_optin) return HJ_ERR_UNSUPPORTED;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess)
-    return HJ_ERR_CUDA;
   const Layout L(a.d, a.N);
   const int tiles = (L.dp / kTI) * (L.Np / kTJ - ((node_shift(a.N) > 0 && !MIX) ? 1 : 0));
   int threads = ((tiles + 31) / 32) * 32;
   if (threads < 64) threads = 64;
   if (threads > 512) threads = 512;
   if (threads < a.d) threads = ((a.d + 31) / 32) * 32;   // x_0 update: one thread per coordinate
+  // groups per CTA: A and the tanh table are shared by a CTA's points, so more of them fit
+  // an SM's shared memory (FP64, d = N = 32: four points against two); no more than one
+  // per SM and CTA while there are fewer points
+  int M = 1;
+  if constexpr (TAB) {
+    const size_t g = L.group_bytes(sizeof(T), MIX);
+    int64_t best = 0;
+    for (int m = 1; m <= kMaxGroups && m * threads <= 512; ++m) {
+      const size_t bytes = smem + (m - 1) * g;
+      if (bytes > (size_t)max_optin || (m > 1 && (int64_t)(m - 1) * nsm >= a.B)) break;
+      const int64_t points = m * (int64_t)((228u * 1024u) / (bytes + 1024));
+      if (points > best) { best = points; M = m; }
+    }
+    smem += (M - 1) * g;
+  }
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+      cudaSuccess)
+    return HJ_ERR_CUDA;
   int bps = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, threads, smem) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, threads * M, smem) != cudaSuccess)
     return HJ_ERR_CUDA;
   if (bps < 1) return HJ_ERR_UNSUPPORTED;
-  const int64_t cap = (int64_t)bps * nsm;
+  const int64_t cap = (int64_t)bps * nsm;         // a point per CTA before a second group's
   const int grid = (int)(a.B < cap ? a.B : cap);
-  kern<<<grid, threads, smem, s>>>(a);
+  kern<<<grid, threads * M, smem, s>>>(a, M);
   return cudaGetLastError() == cudaSuccess ? HJ_OK : HJ_ERR_CUDA;
 }
 
