@@ -271,8 +271,7 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
   if constexpr (MIX) { if (own0) x0xslot[k0] = x0; }
   constexpr int DP = WarpShared<T, F, D, G, MIX, HOPF>::DP;
   constexpr int kLanes = group_lanes<G>();
-  // FP32, one node per lane, up to two warps per point (so that no warp is without a
-  // node), families without a root (F::kBranchFree): the steps run without
+  // FP32, one node per lane, families without a root (F::kBranchFree): the steps run without
   // branches on the node's index.  A lane past node N iterates on values that no other
   // lane reads (node N's lane takes its own p for p_{N+1}); x_j stays where it is for
   // j >= N because p_j - p_{j+1} and the gradient's factor are zero there.  With the
@@ -280,9 +279,12 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
   // went from 190 to 165 instructions per warp and iteration (64 % of the FMA pipe's
   // cycles, as before, are what holds a full GPU): N = 64, FP32, B = 4096 2.34 -> 2.20 ms,
   // B = 1 288 -> 245 us.  20 or more warps per SM (85 registers, no spills) ran 5 %
-  // slower; families whose idle lanes would take a root's rare path, and larger groups,
-  // keep the guards (a guard per warp instead ran the batch 6 % slower).
-  constexpr bool kFree = NPL == 1 && G <= 2 && sizeof(T) == 4 && F::kBranchFree;
+  // slower, and so did a guard per warp inside the step (6 %); families whose idle lanes
+  // would take a root's rare path keep the guards.
+  constexpr bool kFree = NPL == 1 && sizeof(T) == 4 && F::kBranchFree;
+  // G > 2: a warp without any node only keeps the barriers (a loop of its own, so that
+  // the step itself stays one block)
+  const bool warp_on = !kFree || G <= 2 || 1 + wg * 32 <= N;
   [[maybe_unused]] const int pr_lane = jbase < N ? gl + 1 : gl;
   const T taud_x = (!kFree || jbase < N) ? taud : T(0);
 
@@ -489,11 +491,20 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
     T dummy_x = T(0), dummy_p = T(0), dummy_v = T(0);
     // two iterations per trip (FP32, branch-free step): the new x of one is the old x
     // of the next, so fewer registers are copied at the loop's end
+    if (warp_on) {
 #pragma unroll (kFree ? 2 : 1)
-    for (int r = 0; r < plain; ++r)
-      step(std::integral_constant<bool, false>{}, dummy_x, dummy_p, dummy_v);
+      for (int r = 0; r < plain; ++r)
+        step(std::integral_constant<bool, false>{}, dummy_x, dummy_p, dummy_v);
+    } else {
+      for (int r = 0; r < plain; ++r) { group_sync<G>(); group_sync<G>(); }
+    }
     T rx = T(0), rp = T(0), vacc = T(0);
-    step(std::integral_constant<bool, true>{}, rx, rp, vacc);
+    if (warp_on) {
+      step(std::integral_constant<bool, true>{}, rx, rp, vacc);
+    } else {
+      group_sync<G>();
+      group_sync<G>();
+    }
     k_it += plain + 1;
     // each lane's partial (its own nodes, in the iterate type) reduced over the
     // warp by shuffles in that type (a 5-level tree: relative error <= 5 ulp);
