@@ -24,8 +24,8 @@
 // 4 the tiles start at node 1 (node_shift): at d = N = 32 two whole warps of tiles
 // instead of two and a quarter, which cost three.
 // FP64 CTAs hold several groups with a point each, sharing A and the table, so that four
-// points instead of two fit an SM.  d = N = 32, 512 points, FP64: 86.4 -> 56.5 ms, with
-// the groups 52.2.
+// points instead of two fit an SM (the rule at the launch).  d = N = 32, 512 points, FP64:
+// 87 -> 57 ms, with the groups 54.8.
 //
 // MIX = true runs the forward-Euler and trapezoid schemes (HJ_SCHEME_FE/TRAP),
 // H on interval j weighted wR at x_j and wL at x_{j-1}: phase A stores
@@ -438,14 +438,18 @@ hj_status launch_tab(const SolveArgs<T>& a, cudaStream_t s, size_t smem) {
   if (threads < 64) threads = 64;
   if (threads > 512) threads = 512;
   if (threads < a.d) threads = ((a.d + 31) / 32) * 32;   // x_0 update: one thread per coordinate
-  // groups per CTA: A and the tanh table are shared by a CTA's points, so more of them fit
-  // an SM's shared memory (FP64, d = N = 32: four points against two); no more than one
-  // per SM and CTA while there are fewer points
+  // Groups per CTA, where CTAs of one point leave fewer than six warps on an SM (six keep
+  // the FP64 pipe as busy as eight): A and the tanh table are shared by a CTA's points, so
+  // more of them fit (d = N = 32: four points against two, 57.1 -> 54.8 ms for 512 points;
+  // d = 64, N = 24: two against one, 82 -> 58 ms for 300).  With six warps or more,
+  // groups only cost the balance between SMs (d = 20, N = 30, trapezoid, 600 points: 46 ms
+  // without, 53 with).  No more than one point per SM and CTA while there are fewer points.
   int M = 1;
   if constexpr (TAB) {
     const size_t g = L.group_bytes(sizeof(T), MIX);
     int64_t best = 0;
     for (int m = 1; m <= kMaxGroups && m * threads <= 512; ++m) {
+      if (m == 2 && best * (threads / 32) >= 6) break;
       const size_t bytes = smem + (m - 1) * g;
       if (bytes > (size_t)max_optin || (m > 1 && (int64_t)(m - 1) * nsm >= a.B)) break;
       const int64_t points = m * (int64_t)((228u * 1024u) / (bytes + 1024));
