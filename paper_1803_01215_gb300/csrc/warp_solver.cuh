@@ -276,9 +276,9 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
   // lane reads (node N's lane takes its own p for p_{N+1}); x_j stays where it is for
   // j >= N because p_j - p_{j+1} and the gradient's factor are zero there.  With the
   // rows and angles of the quadcopter two-wide and two iterations per trip the loop
-  // went from 190 to 165 instructions per warp and iteration (64 % of the FMA pipe's
-  // cycles, as before, are what holds a full GPU): N = 64, FP32, B = 4096 2.34 -> 2.20 ms,
-  // B = 1 288 -> 245 us.  20 or more warps per SM (85 registers, no spills) ran 5 %
+  // went from 190 to 165 instructions per warp and iteration (a full GPU is held by the FMA
+  // pipe's cycles, 62 %, which two-wide operations do not lower): N = 64, FP32, B = 4096
+  // 2.39 -> 2.24 ms, B = 1 311 -> 261 us.  20 or more warps per SM (85 registers, no spills) ran 5 %
   // slower, and so did a guard per warp inside the step (6 %); families whose idle lanes
   // would take a root's rare path keep the guards.
   constexpr bool kFree = NPL == 1 && sizeof(T) == 4 && F::kBranchFree;
@@ -447,7 +447,8 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
         if constexpr (CHK) {
           T e[D];
           v_sub<T, D>(e, xn, x[i]);
-          rx += v_sumsq<T, D>(e);
+          const T s2 = v_sumsq<T, D>(e);
+          rx += (!kFree || jbase + i < N) ? s2 : T(0);
         }
         if constexpr (CHK && kValueTest) {
           if (a.value_stop && (!kFree || jbase + i < N)) {  // <p_j - p_{j+1}, x_j> - delta H(x_j, p_j)
