@@ -26,12 +26,12 @@
 // FP64 (stop_verdict).  A uniform FP32 batch with N <= 10 runs the instantiation of its
 // N (EXACT): with the per-node guards folded, d = 325 at N = 6 (2659 points) ran
 // 10.1 ms against 25.6 with the guards of the ten-node form.
-// FP32 pipe and two barriers per iteration bound it: a form that kept v_j in the place of
+// The FP32 pipe and two barriers per iteration bound it: a form that kept v_j in the place of
 // z_j, in two-wide operations, with the node sums through shared-memory tiles, took 281
 // instructions per warp and iteration against 436 and no less time (d = 1000, N = 10:
 // 33.8 against 32.1 ms), since a two-wide operation holds the pipe twice as long.
-//  The negative equation (cost_sign = -1) runs the
-// positive one with -g and returns -V and -p, as in Section 6.1.
+// The negative equation (cost_sign = -1) runs the positive one with -g and returns -V
+// and -p, as in Section 6.1.
 #pragma once
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
