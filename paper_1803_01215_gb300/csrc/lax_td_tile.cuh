@@ -278,9 +278,11 @@ lax_td_tile_kernel(const SolveArgs<float> a, int G, int M) {
             const float av = tanhf(acc[r][c]);
             const float zl = (c == 0) ? zL[r] : z[r][c - 1];
             const float v = p[r][c] + sig * (z[r][c] - zl);
-            float pn = (v - lam * av) * ilam;
+            // fused by name: with lam a in both forms below the compiler rounds the product
+            // first, and the two instantiations would not give the same bits
+            float pn = fmaf(-lam, av, v) * ilam;
             if (!LAX1 && HOPF && c == 0 && jt == 0)  // Hopf node 1: prox of sigma g* + lam H
-              pn = __fdividef(v - hc[i0 + r] - lam * av, 1.f + lam + hs[i0 + r]);
+              pn = __fdividef(fmaf(-lam, av, v - hc[i0 + r]), 1.f + lam + hs[i0 + r]);
             if constexpr (CHK) { const float e = pn - p[r][c]; rp += (c <= nup) ? e * e : 0.f; }
             p[r][c] = pn;
             w[c] = (1.f - av * av) * pn;
