@@ -434,6 +434,9 @@ hj_status launch_tile_kernel(const SolveArgs<float>& a, cudaStream_t s) {
   int M = G == 1 ? 4 : G == 2 ? 2 : 1;
   if (TJ == 8 && G <= 4) M = 8 / G;               // eight warps share one copy of A
   while (M > 1 && bytes(M) > (size_t)max_optin) M /= 2;
+  // no second point on an SM while another SM has none (d = 100, N = 32: 152 points take
+  // 6.27 ms two to a CTA, 3.92 one to a CTA; from 153 points on two, 200 points 7.06 ms)
+  while (M > 1 && (int64_t)(M / 2) * nsm >= a.B) M /= 2;
   const size_t smem = bytes(M);
   if (smem > (size_t)max_optin) return HJ_ERR_UNSUPPORTED;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
