@@ -321,9 +321,10 @@ hj_status hj_solve_grad(hj_problem prob, int64_t B, const double* t, int32_t N,
 /* The same gradient, exact for the value after the iterations actually run:
  * reverse-mode differentiation of Algorithm 1's K_b iterations of each point
  * (K_b = iters[b] of the forward solve with the same options), with the
- * iterates (x, p, z) checkpointed every checkpoint_every iterations (at most 64)
- * and each segment between checkpoints run once more during the reverse sweep,
- * its steps kept until they are transposed.  The initial guess x^0 = x + r u and the
+ * iterates (x, p, z) checkpointed every checkpoint_every iterations and each
+ * segment between checkpoints run once more during the reverse sweep, its steps kept
+ * until they are transposed (above 64 iterations in pieces, by further checkpoints
+ * within the one segment at hand).  The initial guess x^0 = x + r u and the
  * pinned x_N = x both carry dV/dx.  At a converged point the result agrees
  * with hj_solve_grad to the stopping accuracy.
  *   xq, t, N, opts   (device, device, host, host) as in the forward solve.
@@ -335,9 +336,12 @@ hj_status hj_solve_grad(hj_problem prob, int64_t B, const double* t, int32_t N,
  * N <= 256, and N <= 128 for the quadcopter in FP64; opts->inner_steps == 1
  * opts->formulation == HJ_FORM_LAX and opts->scheme == HJ_SCHEME_BE
  * (HJ_ERR_UNSUPPORTED otherwise).
- * Allocates a workspace of about 3 (N+1) d (max_iters/checkpoint_every + 1)
- * + 16 N checkpoint_every values per CTA of a grid that fills the GPU (a smaller
- * grid where the device has no room), and synchronises `stream`.
+ * Allocates a workspace per CTA of a grid that fills the GPU (a smaller grid where
+ * the device has no room), and synchronises `stream`.  With C = checkpoint_every (at
+ * most max_iters), S = C up to 64 and max(64, sqrt(C)) above, and L = N rounded up to
+ * 32, 64, 128 or 256, a CTA's values are
+ *   3 (N+1) d (max_iters/C + 1), for C > 64 3 (N+1) d C/S more,
+ *   and S (16 L + 16) (quadcopter) or 16 S (quadratic).
  * Errors: HJ_ERR_INVALID_ARG, HJ_ERR_STEP_SIZE, HJ_ERR_UNSUPPORTED, HJ_ERR_OOM,
  * HJ_ERR_CUDA.                                                               */
 hj_status hj_solve_grad_unrolled(hj_problem prob, int64_t B, const double* xq, const double* t,

@@ -13,7 +13,11 @@
 //             needs in a history buffer, and then for k = last .. first the
 //             transposed Jacobian of step k is applied to the adjoint (xbar, pbar,
 //             zbar), accumulating parameter adjoints.  2 K forward and K
-//             transposed steps per point.
+//             transposed steps per point.  The history holds S = C steps up to
+//             C = 64; a longer segment is run once with checkpoints every S steps
+//             and then by these, as a segment is by its own: 3 K forward steps, and
+//             the workspace stays the K / C checkpoints that were asked for, C / S
+//             more and S steps.
 // At a converged point this equals the envelope gradient of hj_solve_grad.
 // One CTA of G warps per point (lane l <-> node l + 1; lanes 0..D-1 also hold one
 // coordinate each of node 0); neighbour terms go through per-lane shared-memory
@@ -465,12 +469,15 @@ __global__ void __launch_bounds__(32 * G) adjoint_kernel(const AdjArgs<T> a) {
       }
     };
 
-    // ---- forward with checkpoints; the last segment leaves its history at once
-    const int nseg = (K + a.C - 1) / a.C;
-    const int klast = (nseg - 1) * a.C;             // first iteration of the last segment
-    for (int k = 0; k < K; ++k) {
-      if (k % a.C == 0 && k < klast) save(k / a.C);
-      step(k >= klast ? hist + (size_t)(k - klast) * hrow : nullptr);
+    // ---- forward with checkpoints; the last piece (up to S steps) of the last segment
+    // leaves its history at once.  kb: first iteration of the segment at hand, ks: of
+    // the piece whose history is in the buffer.
+    int kb = K > 0 ? (K - 1) / a.C * a.C : 0;
+    int ks = K > 0 ? kb + (K - 1 - kb) / a.S * a.S : 0;
+    for (int k = 0, next = 0, slot = 0, gap = a.C; k < K; ++k) {   // next: that of the next checkpoint
+      if (k == kb) { next = kb; slot = a.slot_s; gap = a.S; }
+      if (k == next && k < ks) { save(slot++); next += gap; }
+      step(k >= ks ? hist + (size_t)(k - ks) * hrow : nullptr);
     }
     __syncthreads();
 
@@ -521,17 +528,27 @@ __global__ void __launch_bounds__(32 * G) adjoint_kernel(const AdjArgs<T> a) {
       }
     }
 
-    // ---- backward sweep, newest segment first
-    for (int sgi = nseg - 1; sgi >= 0; --sgi) {
-      const int kb = sgi * a.C;
-      const int n = min(K - kb, a.C);
+    // ---- backward sweep, newest piece first; kend: the iterations not yet transposed
+    for (int kend = K; kend > 0; kend = ks) {
       __syncthreads();                                // the slots are free again
-      if (sgi < nseg - 1) {
-        load(sgi);
-        for (int r = 0; r < n; ++r) step(hist + (size_t)r * hrow);
+      if (kend < K) {
+        int k, next = kend, slot = a.slot_s;
+        if (ks > kb) {                                // the piece before, of the same segment
+          k = ks -= a.S;
+          load(a.slot_s + (ks - kb) / a.S);
+        } else {                                      // the last piece of the segment before
+          k = next = kb -= a.C;
+          ks = kb + (a.C - 1) / a.S * a.S;
+          load(kb / a.C);
+        }
+        for (; k < kend; ++k) {
+          if (k == next && k < ks) { save(slot++); next += a.S; }
+          step(k >= ks ? hist + (size_t)(k - ks) * hrow : nullptr);
+        }
         __syncthreads();
       }
-      auto fetch = [&](int r, int buf) {              // history of the segment's step r
+      const int n = kend - ks;
+      auto fetch = [&](int r, int buf) {              // history of the piece's step r
         if constexpr (FAM == 1) {
           if (mine) {
             const char* s = reinterpret_cast<const char*>(hist + (size_t)r * hrow) + 16 * gl;
@@ -703,6 +720,8 @@ __global__ void __launch_bounds__(32 * G) adjoint_kernel(const AdjArgs<T> a) {
   }
 }
 
+constexpr int kHistSteps = 64;
+
 // Everything a launch of one instantiation needs: kernel, threads, shared memory,
 // and the workspace of one CTA for (K_cap, C).
 template <typename T, int FAM, int D, int G>
@@ -720,10 +739,19 @@ hj_status launch_adj_g(AdjArgs<T>& a, cudaStream_t s) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * G, smem) != cudaSuccess)
       return HJ_ERR_CUDA;
-    const size_t ckpt = ((size_t)(a.K_cap / a.C + 1) * 3 * (a.N + 1) * D + 15) / 16 * 16;
+    // steps whose history is kept: the whole segment up to 64 (C is not above K_cap here),
+    // beyond that 64, or about sqrt(C) where checkpoints every 64 steps would be the more
+    a.S = a.C;
+    if (a.C > kHistSteps) {
+      a.S = kHistSteps;
+      while ((int64_t)a.S * a.S < a.C) ++a.S;
+    }
+    a.slot_s = a.K_cap / a.C + 1;
+    const int n_s = a.S < a.C ? (a.C - 1) / a.S + 1 : 0;
+    const size_t ckpt = (((size_t)a.slot_s + n_s) * 3 * (a.N + 1) * D + 15) / 16 * 16;
     const size_t hrow = (size_t)32 * G * hist_vals<FAM>() + 16;
     a.hist_off = ckpt;
-    a.work_per_cta = ckpt + (size_t)(a.C < a.K_cap ? a.C : (a.K_cap > 0 ? a.K_cap : 1)) * hrow;
+    a.work_per_cta = ckpt + (size_t)a.S * hrow;
     int64_t grid = (int64_t)nsm * (per_sm > 0 ? per_sm : 1);
     if (a.B < grid) grid = a.B;
     // fewer CTAs where the device has no room for all of them
@@ -761,15 +789,10 @@ hj_status launch_adj(AdjArgs<T>& a, cudaStream_t s) {
 
 }  // namespace
 
-// Segments longer than this are cut: the history of a segment is kept in the
-// workspace, so a long one would hold many steps (checkpoint_every asks for at most
-// this many iterations between checkpoints).
-constexpr int kMaxSegment = 64;
-
 template <typename T>
 hj_status launch_adjoint(int family, const AdjArgs<T>& args, cudaStream_t s) {
   AdjArgs<T> a = args;
-  if (a.C > kMaxSegment) a.C = kMaxSegment;
+  if (a.C > a.K_cap) a.C = a.K_cap > 0 ? a.K_cap : 1;   // one segment either way
   if (a.N < 1 || a.N > 256) return HJ_ERR_UNSUPPORTED;
   if (family == HJ_FAMILY_QUADCOPTER && a.d == 12) return launch_adj<T, 1, 12>(a, s);
   if (family == HJ_FAMILY_QUADRATIC) {
