@@ -145,8 +145,8 @@ __device__ __forceinline__ void qc_dHdpar(const QCNode<T>& n, const QCPar& q, co
 // A sum over iterations.  FP64 terms are added in FP64.  FP32 terms are added into
 // three floats by Knuth's error-free TwoSum (the rounding error of the first sum
 // goes into the second, the second's into the third), which is folded into an FP64
-// sum after every segment: within 64 steps of 3 terms the three floats hold the sum
-// to 192^3 2^-72 of it, under the 192 2^-53 that adding the converted terms in FP64
+// sum after 64 steps at most: within 64 steps of 4 terms (a_h) the three floats hold the
+// sum to 256^3 2^-72 of it, under the 256 2^-53 that adding the converted terms in FP64
 // would give, and every instruction runs on the FP32 pipe.
 template <typename T>
 struct StepSum {
@@ -276,6 +276,8 @@ __device__ __forceinline__ void qc_gradx_vjp(const QCNode<T>& n, const QCPar& q,
     xb[3 + k] += acc;
   }
 }
+
+constexpr int kHistSteps = 64;   // steps whose history is kept, and which a StepSum adds, at most
 
 // 16-byte asynchronous copy global -> shared (a thread's own data: no barrier)
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
@@ -675,11 +677,13 @@ __global__ void __launch_bounds__(32 * G) adjoint_kernel(const AdjArgs<T> a) {
 #pragma unroll
         for (int kk = 0; kk < D; ++kk) { xb[kk] = nxb[kk]; pb[kk] = npb[kk]; zb[kk] = nzb[kk]; }
         x0p = x0p_next;
-      }
-      if constexpr (FAM == 1) {
-        QCSums& q = sh.sums[gl];
-        q.ma += steps.ma.take(); q.mc += steps.mc.take(); q.ah += steps.ah.take();
-        q.gz += steps.gz.take(); q.eps += steps.eps.take();
+        if constexpr (FAM == 1) {
+          if (r % kHistSteps == 0) {                  // StepSum's bound is for 64 steps
+            QCSums& q = sh.sums[gl];
+            q.ma += steps.ma.take(); q.mc += steps.mc.take(); q.ah += steps.ah.take();
+            q.gz += steps.gz.take(); q.eps += steps.eps.take();
+          }
+        }
       }
     }
 
@@ -719,8 +723,6 @@ __global__ void __launch_bounds__(32 * G) adjoint_kernel(const AdjArgs<T> a) {
     }
   }
 }
-
-constexpr int kHistSteps = 64;
 
 // Everything a launch of one instantiation needs: kernel, threads, shared memory,
 // and the workspace of one CTA for (K_cap, C).

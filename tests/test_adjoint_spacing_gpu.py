@@ -48,3 +48,11 @@ def test_spacing_bounds_the_workspace():
     w = W.quadcopter(B=3, seed=3, N=128, t=0.4)
     w["iters"] = np.array([5, 70, 140])
     _same(_grad(w, "fp32", 1_000_000, 2_000_000_000), _grad(w, "fp32", 1, 140))
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_pieces_longer_than_64_steps(precision):
+    """Checkpoints every 1e6 iterations: pieces of 1000 steps, the parameter sums folded every 64."""
+    w = W.quadcopter(B=4, seed=3, N=20, t=0.4)
+    w["iters"] = np.array([64, 65, 700, 1001])
+    _same(_grad(w, precision, 1_000_000, 1_000_000), _grad(w, precision, 1, 1001))
