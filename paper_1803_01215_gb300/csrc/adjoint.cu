@@ -147,7 +147,8 @@ __device__ __forceinline__ void qc_dHdpar(const QCNode<T>& n, const QCPar& q, co
 // goes into the second, the second's into the third), which is folded into an FP64
 // sum after 64 steps at most: within 64 steps of 4 terms (a_h) the three floats hold the
 // sum to 256^3 2^-72 of it, under the 256 2^-53 that adding the converted terms in FP64
-// would give, and every instruction runs on the FP32 pipe.
+// would give, and every instruction runs on the FP32 pipe.  The callers add only terms
+// below 2^118 this way, so that no sum of 256 overflows, and larger ones to FP64 (wide).
 template <typename T>
 struct StepSum {
   double s = 0.0;
@@ -165,15 +166,25 @@ struct StepSum<float> {
   }
   __device__ __forceinline__ void add(float t) { c = __fadd_rn(c, two_sum(b, two_sum(a, t))); }
   __device__ __forceinline__ double take() {
-    // an overflowed sum stays as it is (its error terms are not numbers)
-    const double r = isfinite(a) ? (double)a + ((double)b + (double)c) : (double)a;
+    const double r = (double)a + ((double)b + (double)c);
     a = b = c = 0.f;
     return r;
   }
 };
 
+// Whether one of the terms is too large for a StepSum (a NaN is not: it stays one there).
+template <typename... U>
+__device__ __forceinline__ bool wide(float t, U... ts) {
+  float m = fabsf(t);
+  ((m = fmaxf(m, fabsf(ts))), ...);
+  return m >= 0x1p118f;
+}
+template <typename... U>
+__device__ __forceinline__ bool wide(double, U...) { return false; }
+
 // Sums over the iterations that the parameter adjoints are linear in; the constant
 // factors are applied once per point (qc_par).
+// big: the lane's FP64 sums.
 template <typename T>
 struct QCStep { StepSum<T> ma, mc, ah, gz, eps; };
 struct QCSums { double ma, mc, ah, gz, eps; };
@@ -190,7 +201,7 @@ template <typename T>
 __device__ __forceinline__ void qc_prox_vjp(const QCNode<T>& n, const QCPar& q, T L,
                                             const T (&v)[12], const T (&pp)[12],
                                             const T (&pb)[12], T (&vb)[12], T (&xb)[12],
-                                            QCStep<T>& par) {
+                                            QCStep<T>& par, QCSums& big) {
   const T al = T(1) + L * T(q.eps), ial = T(1) / al, irate = T(1) / (al + L);
   const T m = T(q.m), minv = T(1) / m;
   T alb = T(0);
@@ -227,18 +238,26 @@ __device__ __forceinline__ void qc_prox_vjp(const QCNode<T>& n, const QCPar& q, 
     bbar[r] += bwb * w[r] + T(2) * bbb * b[r];
     wb[r] += bwb * b[r];
   }
-  T ab[3];
+  T ab[3], tm[3], ta[3];
   for (int r = 0; r < 3; ++r) {
     ab[r] = bbar[r] * minv;
-    par.ma.add(bbar[r] * n.a[r]);
+    tm[r] = bbar[r] * n.a[r];
     vb[6 + r] += wb[r];
     ab[r] += -L * T(q.ah) * wb[r];
-    par.ah.add(-(L * wb[r] * n.a[r]));
+    ta[r] = -(L * wb[r] * n.a[r]);
   }
-  par.gz.add(L * wb[2]);
+  const T tg = L * wb[2], te = L * alb;           // al = 1 + L eps
+  if (!wide(tm[0], tm[1], tm[2], ta[0], ta[1], ta[2], tg, te)) {
+    for (int r = 0; r < 3; ++r) { par.ma.add(tm[r]); par.ah.add(ta[r]); }
+    par.gz.add(tg);
+    par.eps.add(te);
+  } else {
+    for (int r = 0; r < 3; ++r) { big.ma += (double)tm[r]; big.ah += (double)ta[r]; }
+    big.gz += (double)tg;
+    big.eps += (double)te;
+  }
   for (int c = 0; c < 3; ++c)
     xb[3 + c] += n.J[c] * ab[0] + n.J[3 + c] * ab[1] + n.J[6 + c] * ab[2];
-  par.eps.add(L * alb);                           // al = 1 + L eps
 }
 
 // Reverse of qc_gradx: given gb = dL/dg, add dL/dx (angles) to xb, dL/dp to pb,
@@ -246,7 +265,7 @@ __device__ __forceinline__ void qc_prox_vjp(const QCNode<T>& n, const QCPar& q, 
 template <typename T>
 __device__ __forceinline__ void qc_gradx_vjp(const QCNode<T>& n, const QCPar& q, const T (&p)[12],
                                              const T (&gb)[12], T (&xb)[12], T (&pb)[12],
-                                             QCStep<T>& par) {
+                                             QCStep<T>& par, QCSums& big) {
   const T minv = T(1.0 / q.m);
   for (int k = 0; k < 3; ++k) { pb[k] += gb[6 + k]; pb[3 + k] += gb[9 + k]; }
   T qv[3] = {p[6], p[7], p[8]};
@@ -263,9 +282,14 @@ __device__ __forceinline__ void qc_gradx_vjp(const QCNode<T>& n, const QCPar& q,
     qb[r] = n.J[3 * r] * hb[0] + n.J[3 * r + 1] * hb[1] + n.J[3 * r + 2] * hb[2];
     for (int c = 0; c < 3; ++c) Jb[3 * r + c] = qv[r] * hb[c];
   }
-  par.ah.add(coefb);
-  const T sb = coefb * minv * minv;
-  par.mc.add(s * coefb);
+  const T sb = coefb * minv * minv, tc = s * coefb;
+  if (!wide(coefb, tc)) {
+    par.ah.add(coefb);
+    par.mc.add(tc);
+  } else {
+    big.ah += (double)coefb;
+    big.mc += (double)tc;
+  }
   T ab[3];
   for (int r = 0; r < 3; ++r) { ab[r] = sb * qv[r]; qb[r] += sb * n.a[r]; }
   for (int r = 0; r < 3; ++r) pb[6 + r] += qb[r];
@@ -608,7 +632,8 @@ __global__ void __launch_bounds__(32 * G) adjoint_kernel(const AdjArgs<T> a) {
           for (int kk = 0; kk < D; ++kk) gb[kk] = taud * xpb[kk];
           if constexpr (FAM == 1)
             qc_gradx_vjp<T>(nd, qp, reinterpret_cast<const T(&)[12]>(pn), reinterpret_cast<const T(&)[12]>(gb),
-                            reinterpret_cast<T(&)[12]>(nxb), reinterpret_cast<T(&)[12]>(pnb), steps);
+                            reinterpret_cast<T(&)[12]>(nxb), reinterpret_cast<T(&)[12]>(pnb), steps,
+                            sh.sums[gl]);
         } else {
 #pragma unroll
           for (int kk = 0; kk < D; ++kk) xpb[kk] = T(0);
@@ -653,7 +678,7 @@ __global__ void __launch_bounds__(32 * G) adjoint_kernel(const AdjArgs<T> a) {
           if constexpr (FAM == 1)
             qc_prox_vjp<T>(nd, qp, L, reinterpret_cast<const T(&)[12]>(v), reinterpret_cast<const T(&)[12]>(pn),
                            reinterpret_cast<const T(&)[12]>(pnb), reinterpret_cast<T(&)[12]>(vb),
-                           reinterpret_cast<T(&)[12]>(nxb), steps);
+                           reinterpret_cast<T(&)[12]>(nxb), steps, sh.sums[gl]);
           else
 #pragma unroll
             for (int kk = 0; kk < D; ++kk) vb[kk] = pnb[kk] / (T(1) + L);
