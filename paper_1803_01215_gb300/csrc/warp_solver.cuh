@@ -101,9 +101,12 @@ struct grad_from<F, std::void_t<decltype(F::kGradFrom)>> : std::integral_constan
 // lanes of this thread's 16-lane half
 __device__ __forceinline__ unsigned half_mask() { return 0xFFFFu << (threadIdx.x & 16); }
 
+// Barrier of a group.  G > 1: the CTA's G warps by a barrier that counts their threads,
+// since they may wait at different places of the program (a warp without a node runs a
+// loop of its own), which __syncthreads does not allow; each warp is uniform.
 template <int G>
 __device__ __forceinline__ void group_sync() {
-  if constexpr (G > 1) __syncthreads();
+  if constexpr (G > 1) asm volatile("bar.sync 1, %0;" ::"n"(32 * G) : "memory");
   else if constexpr (G == 1) __syncwarp();
   else __syncwarp(half_mask());
 }
