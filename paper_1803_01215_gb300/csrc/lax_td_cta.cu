@@ -443,7 +443,7 @@ hj_status launch_tab(const SolveArgs<T>& a, cudaStream_t s, size_t smem) {
   // more of them fit (d = N = 32: four points against two, 57.1 -> 54.8 ms for 512 points;
   // d = 64, N = 24: two against one, 82 -> 58 ms for 300).  With six warps or more,
   // groups only cost the balance between SMs (d = 20, N = 30, trapezoid, 600 points: 46 ms
-  // without, 53 with).  No more than one point per SM and CTA while there are fewer points.
+  // without, 53 with).  No m-th group while m - 1 points per SM take the whole batch.
   int M = 1;
   if constexpr (TAB) {
     const size_t g = L.group_bytes(sizeof(T), MIX);
@@ -464,7 +464,9 @@ hj_status launch_tab(const SolveArgs<T>& a, cudaStream_t s, size_t smem) {
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, threads * M, smem) != cudaSuccess)
     return HJ_ERR_CUDA;
   if (bps < 1) return HJ_ERR_UNSUPPORTED;
-  const int64_t cap = (int64_t)bps * nsm;         // a point per CTA before a second group's
+  // CTAs for all points, though a CTA of M groups takes M: the groups draw as they start, so
+  // where points run out the last CTAs get none and end at once
+  const int64_t cap = (int64_t)bps * nsm;
   const int grid = (int)(a.B < cap ? a.B : cap);
   kern<<<grid, threads * M, smem, s>>>(a, M);
   return cudaGetLastError() == cudaSuccess ? HJ_OK : HJ_ERR_CUDA;
