@@ -76,7 +76,9 @@ __device__ __forceinline__ float tanh_c<float>(float y, const double*) { return 
 
 // Node j of a point with N steps is column j + node_shift(N) of the state arrays: for
 // N a multiple of 4 the nodes 1..N fill whole 4-column tiles and node 0 sits in the
-// last column of a tile of its own (the products skip it, mixed schemes apart).
+// last column of a tile of its own, which the products skip.  The mixed schemes need node
+// 0's products and keep node j in column j: d = N = 32, 300 points, FP32, forward Euler
+// take 4.67 ms so and 4.98 shifted.
 __host__ __device__ inline int node_shift(int N) { return N % 4 == 0 ? 3 : 0; }
 
 struct Layout {
@@ -166,8 +168,8 @@ lax_td_cta_kernel(const SolveArgs<T> a, int M) {
       continue;
     }
     const int Np = round4(N + 1);
-    const int sh = node_shift(N);                          // node j: column j + sh
-    const int jt0 = (sh > 0 && !MIX) ? 1 : 0;              // first tile the products run on
+    const int sh = MIX ? 0 : node_shift(N);                // node j: column j + sh
+    const int jt0 = sh > 0 ? 1 : 0;                        // first tile the products run on
     const int tilesI = dp / kTI, tilesJ = Np / kTJ - jt0;
     const int ntiles = tilesI * tilesJ;
     const double delta = a.t[b] / N;                      // value epilogue only
