@@ -754,7 +754,7 @@ __global__ void __launch_bounds__(32 * G) adjoint_kernel(const AdjArgs<T> a) {
 template <typename T, int FAM, int D, int G>
 hj_status launch_adj_g(AdjArgs<T>& a, cudaStream_t s) {
   using Sh = AdjShared<T, FAM, D, G>;
-  // FP64 12-D lanes of 256 nodes stay refused (their slots alone exceed 48 KB)
+  // FP64 quadcopter beyond 128 nodes: outside the entry point's range, not built
   if constexpr (sizeof(T) == 8 && D == 12 && G == 8) {
     return HJ_ERR_UNSUPPORTED;
   } else {

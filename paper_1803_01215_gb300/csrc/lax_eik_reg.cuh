@@ -25,7 +25,10 @@
 // as double-floats (FP32 iterates: as accurate as FP64, on the FP32 pipe) or in
 // FP64 (stop_verdict).  A uniform FP32 batch with N <= 10 runs the instantiation of its
 // N (EXACT): with the per-node guards folded, d = 325 at N = 6 (2659 points) ran
-// 10.1 ms against 25.6 with the guards of the ten-node form.
+// 10.1 ms against 25.6 with the guards of the ten-node form.  For N <= 9 it sums in the
+// guarded form's order, so a uniform batch and a ragged plan give the same bits; for
+// N = 10 the unguarded form has always had an order of its own, and the two differ in the
+// last bits.
 // The FP32 pipe and two barriers per iteration bound it: a form that kept v_j in the place of
 // z_j, in two-wide operations, with the node sums through shared-memory tiles, took 281
 // instructions per warp and iteration against 436 and no less time (d = 1000, N = 10:

@@ -13,7 +13,10 @@ namespace {
 // Warps a point takes with j-tiles in whole blocks of four, rounded up to a power of two:
 // up to 8 with eight-node tiles (about 240 registers), 16 with four-node tiles (128
 // registers); 0 if it does not fit.  This is the range of (d, N) that the kernel serves;
-// the launch itself takes as many warps as the tiles fill.
+// the launch itself takes as many warps as the tiles fill.  It is not the largest that
+// would fit (d = 100, N = 65..80 fills 8 warps of eight-node tiles and is left to the
+// shared-memory kernel, whose sums round in another order): points served by either
+// kernel give the bits that they always gave.
 int group_warps(int d, int N, int TJ) {
   const int TIc = (d + 3) / 4, TJc = (N + TJ - 1) / TJ;
   const int w = (4 * TIc * ((TJc + 3) / 4) + 31) / 32;

@@ -74,14 +74,6 @@ __device__ __forceinline__ void group_barrier(int grp, int G) {
 }
 
 template <int TJ>
-__device__ __forceinline__ void loadv(const float* p, float (&v)[TJ]) {
-#pragma unroll
-  for (int q = 0; q < TJ / 4; ++q) {
-    const float4 a = *reinterpret_cast<const float4*>(p + 4 * q);
-    v[4 * q] = a.x; v[4 * q + 1] = a.y; v[4 * q + 2] = a.z; v[4 * q + 3] = a.w;
-  }
-}
-template <int TJ>
 __device__ __forceinline__ void storev(float* p, const float (&v)[TJ]) {
 #pragma unroll
   for (int q = 0; q < TJ / 4; ++q)

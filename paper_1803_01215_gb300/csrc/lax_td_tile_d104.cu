@@ -1,4 +1,9 @@
 // Register-tiled tanh-drift kernel, d <= 104: tiles of 8 nodes.
+// A row stride of A below 128 leaves shared memory for more points where the groups are
+// one warp: d = 72, N = 8 eight of them beside A against four (8000 points: 6.64 ms,
+// 7.77 with the stride 128; d = 70, N = 7 5.86 and 6.98).  From N = 9 on, and above d =
+// 72, the two strides measured the same (d = 72..104, N = 8..96): the class could end
+// anywhere between.
 #include "lax_td_tile.cuh"
 
 namespace hj {

@@ -281,12 +281,16 @@ __device__ __forceinline__ void solve_point(const SolveArgs<T>& a, const F& fam,
   // rows and angles of the quadcopter two-wide and two iterations per trip the loop
   // went from 190 to 165 instructions per warp and iteration (a full GPU is held by the FMA
   // pipe's cycles, 62 %, which two-wide operations do not lower): N = 64, FP32, B = 4096
-  // 2.39 -> 2.24 ms, B = 1 311 -> 261 us.  20 or more warps per SM (85 registers, no spills) ran 5 %
+  // 2.39 -> 2.24 ms, B = 1 311 -> 261 us (whole calls with the certificate, passes back to
+  // back).  20 or more warps per SM (85 registers, no spills) ran 5 %
   // slower, and so did a guard per warp inside the step (6 %); families whose idle lanes
   // would take a root's rare path keep the guards.
   constexpr bool kFree = NPL == 1 && sizeof(T) == 4 && F::kBranchFree;
   // G > 2: a warp without any node only keeps the barriers (a loop of its own, so that
-  // the step itself stays one block)
+  // the step itself stays one block).  G = 2 has such a warp only where the caller asks for
+  // two warps at N <= 32 (N = 30, 2000 points 636 us, 603 with the second loop, 675 with
+  // guards); the second loop costs every N in 33..64 at small batches (B = 1, N = 64
+  // 261 -> 287 us), so it is left out.
   const bool warp_on = !kFree || G <= 2 || 1 + wg * 32 <= N;
   [[maybe_unused]] const int pr_lane = jbase < N ? gl + 1 : gl;
   const T taud_x = (!kFree || jbase < N) ? taud : T(0);
