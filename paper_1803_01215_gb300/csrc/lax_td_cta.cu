@@ -20,7 +20,7 @@
 // FP64 iterates are bound by the FP64 pipe (80 % busy: one instruction holds a
 // sub-partition's pipe about 64 cycles per warp), so what counts is the FP64
 // instructions per element: 70 of them were CUDA's tanh (both of its ranges, for a warp
-// whose lanes differ), 15 are the Taylor table's (tanh64.cuh); and for N a multiple of
+// whose lanes differ), 13 are the Taylor table's (tanh64.cuh); and for N a multiple of
 // 4 the tiles start at node 1 (node_shift): at d = N = 32 two whole warps of tiles
 // instead of two and a quarter, which cost three.
 // FP64 CTAs hold several groups with a point each, sharing A and the table, so that four

@@ -1,4 +1,4 @@
-// tanh of an FP64 argument in 15 FP64 instructions, without a branch: Taylor's
+// tanh of an FP64 argument in 13 FP64 instructions, without a branch: Taylor's
 // expansion about the nearest multiple of 1/16 from a table of its coefficients.
 //
 // tanh' = 1 - tanh^2 gives every coefficient from the first: with t = sum c_n b^n,
@@ -10,7 +10,10 @@
 // arithmetic on the host against 113-bit values at 6e6 arguments.  CUDA's tanh, measured
 // the same way, is off by 1.40 ulp at most (at 0.549).  With c_0 one double from a
 // tanh call, and the sum folded into it by one multiply-add, the table's largest error
-// was 1.3 to 1.9 ulp in 13 instructions.  From 19.0625 on tanh rounds to 1.
+// was 1.3 to 1.9 ulp, in 13 instructions too: the two more for the sum are won back by
+// finding the row in FP32 and integer instructions, which do not wait for the FP64 pipe
+// (d = 8, N = 10, 400 points: 6.11 ms with the one-double table, 6.36 with the row found
+// in FP64, 5.93 so; d = N = 40, 160 points 71.0, 72.2 and 69.9).  From 19.0625 on tanh rounds to 1.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -63,9 +66,15 @@ __device__ __forceinline__ double tanh_taylor(double x, const double* tab) {
   // |x| capped at 19.0625 by its bits; NaN is returned as it came (below)
   const bool big = ahi >= 0x40331000;
   const double ax = __hiloint2double(big ? 0x40331000 : ahi, big ? 0 : lo);
-  const double t = fma(ax, 16.0, 0x1.8p52);          // nearest multiple of 1/16 in the low word
-  const double b = fma(t - 0x1.8p52, -0.0625, ax);   // exact
-  const double2* c = reinterpret_cast<const double2*>(tab + __double2loint(t) * kTanhRow);
+  // k / 16, the nearest multiple (to |x|'s upper 20 bits), in FP32 and integer
+  // instructions: |x| as a float, 0 below 2^-127; k in the low bits of 1.5 2^23 + 16 |x|;
+  // k as a float, and its bits as those of the double k / 16
+  const int fi = max((big ? 0x40331000 : ahi) - (896 << 20), 0) << 3;
+  const float m = fmaf(__int_as_float(fi), 16.0f, 12582912.0f);
+  const int k = __float_as_int(m) - 0x4b400000;
+  const int ci = (__float_as_int(m - 12582912.0f) >> 3) + (892 << 20);
+  const double b = ax - __hiloint2double(k == 0 ? 0 : ci, 0);   // exact
+  const double2* c = reinterpret_cast<const double2*>(tab + k * kTanhRow);
   const double2 c0 = c[0], c2 = c[1], c4 = c[2], c6 = c[3], c8 = c[4], c10 = c[5];
   double r = fma(c10.x, b, c8.y);
   r = fma(r, b, c8.x);
