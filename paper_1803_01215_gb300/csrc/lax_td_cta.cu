@@ -25,7 +25,7 @@
 // instead of two and a quarter, which cost three.
 // FP64 CTAs hold several groups with a point each, sharing A and the table, so that four
 // points instead of two fit an SM (the rule at the launch).  d = N = 32, 512 points, FP64:
-// 87 -> 57 ms, with the groups 54.8.
+// 87 -> 57 ms, with the groups 55.4.
 //
 // MIX = true runs the forward-Euler and trapezoid schemes (HJ_SCHEME_FE/TRAP),
 // H on interval j weighted wR at x_j and wL at x_{j-1}: phase A stores

@@ -6,14 +6,15 @@
 // leave a remainder below 2^-61 (|c_11| <= 0.0089, its largest in the first row, where
 // it is 2^-56 of the result).  c_0 is a pair of doubles, good to 2^-100, so what is left
 // is the rounding of the last addition, of c_1 b and of c_1: 0.87 ulp at most (at
-// 0.0313, where c_1 b and the result are of one size) and 0.70 from 0.16 on, by the same
+// 0.0313, where c_1 b and the result are of one size) and 0.64 from 0.1 on, by the same
 // arithmetic on the host against 113-bit values at 6e6 arguments.  CUDA's tanh, measured
 // the same way, is off by 1.40 ulp at most (at 0.549).  With c_0 one double from a
 // tanh call, and the sum folded into it by one multiply-add, the table's largest error
 // was 1.3 to 1.9 ulp, in 13 instructions too: the two more for the sum are won back by
 // finding the row in FP32 and integer instructions, which do not wait for the FP64 pipe
 // (d = 8, N = 10, 400 points: 6.11 ms with the one-double table, 6.36 with the row found
-// in FP64, 5.93 so; d = N = 40, 160 points 71.0, 72.2 and 69.9).  From 19.0625 on tanh rounds to 1.
+// in FP64, 5.93 so; d = N = 40, 160 points 71.0, 72.2 and 69.9).  From 19.0625 on tanh
+// rounds to 1.
 #pragma once
 #include <cuda_runtime.h>
 
