@@ -25,7 +25,7 @@
 // copied to shared memory by cp.async while step k is transposed.
 // Families: quadratic (d <= 4) and quadcopter (d = 12).
 //
-// What bounds it: instruction issue at 8 warps per SM (248 registers; about 1100
+// What bounds it: instruction issue at 8 warps per SM (255 registers; about 1100
 // instructions per warp and iteration, 2 forward steps and a transposed one).
 // Rebuilding s^k from its checkpoint for every k cost K C / 2 forward steps; with the
 // history a segment is run once, in 64 bytes per lane and step that mostly stay in
